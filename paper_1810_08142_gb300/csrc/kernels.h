@@ -88,6 +88,8 @@ struct CrtOut {
 // enough (the product then runs in blocks of K, each added in FP64, and of
 // rows), down to the figure for m = 128, n = 16, K = 8192
 size_t crt_gemm_bytes(long long m, long long n, long long K, int sms);
+// rows, columns and K of the blocks that crt_gemm (m >= n) takes in this scratch; false: none fits
+bool crt_gemm_blocks(long long m, long long n, long long K, int sms, size_t scratch_bytes, long long (&blk)[3]);
 cudaError_t crt_init_attributes();  // once per device, outside stream capture
 cudaError_t crt_gemm(const CrtView &A, const CrtView &B, const CrtOut &C, double alpha, double beta, void *scratch,
                      size_t scratch_bytes, int *status, int sms, cudaStream_t s);

@@ -1,0 +1,62 @@
+"""Blocks of the FP64-class product (csrc/crt_gemm.cu) against its scratch: what
+every block lays out, counted here from the documented layout, fits, for any
+shape and any scratch down to the least one.  No device."""
+import ctypes
+import random
+
+import pytest
+
+MODULI = 16
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_1810_08142_gb300 import build
+    return ctypes.CDLL(build.build())
+
+
+def up(x, to):
+    return (x + to - 1) // to * to
+
+
+def block_need(m, n, k):
+    """Residues (2 bytes) and exponents of both operands, one byte per modulus, row and padded column."""
+    kp = up(k, 8)
+    return sum(up(MODULI * r * kp * 2, 256) + up(4 * r, 256) for r in (m, n)) + MODULI * m * up(n, 16)
+
+
+def blocks(lib, m, n, k, scratch, sms=152):
+    f = getattr(lib, "_ZN6ladder15crt_gemm_blocksExxximRA3_x")
+    f.restype = ctypes.c_bool
+    f.argtypes = [ctypes.c_longlong] * 3 + [ctypes.c_int, ctypes.c_size_t, ctypes.POINTER(ctypes.c_longlong * 3)]
+    out = (ctypes.c_longlong * 3)()
+    return list(out) if f(m, n, k, sms, scratch, ctypes.byref(out)) else None
+
+
+def check(lib, m, n, k, scratch):
+    b = blocks(lib, m, n, k, scratch)
+    assert b is not None, (m, n, k, scratch)
+    for x, whole, step in zip(b, (m, n, k), (128, 16, 64)):
+        assert 0 < x <= whole and (x == whole or x % step == 0)
+    # the full blocks and the last ones of every direction
+    tails = [(x, (whole - 1) % x + 1) for x, whole in zip(b, (m, n, k))]
+    for mm in tails[0]:
+        for nn in tails[1]:
+            for kk in tails[2]:
+                assert block_need(mm, nn, kk) <= scratch, (m, n, k, scratch, b)
+
+
+# the (kc|ld) product of a dressed ladder, m = n = o v, in 1 GiB of scratch
+@pytest.mark.parametrize("o,v,n", [(20, 406, 1380), (26, 319, 1276), (15, 447, 2155), (17, 417, 1950), (34, 259, 1036),
+                                   (23, 362, 1267)])
+def test_rows_halved_below_the_columns(lib, o, v, n):
+    check(lib, o * v, o * v, n, 1 << 30)
+
+
+def test_every_scratch_down_to_the_least(lib):
+    rng = random.Random(1)
+    least = block_need(128, 16, 8192)
+    for _ in range(4000):
+        m, n = sorted((int(2 ** rng.uniform(0, 17)), int(2 ** rng.uniform(0, 17))), reverse=True)
+        check(lib, m, n, int(2 ** rng.uniform(0, 18)), int(least * 2 ** rng.uniform(0, 8)) + 256)
+    assert blocks(lib, 128, 16, 8192, least - 256) is None

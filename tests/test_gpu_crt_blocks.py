@@ -1,0 +1,21 @@
+"""The FP64-class product (csrc/crt_gemm.cu) in blocks of fewer rows than columns."""
+import pytest
+
+from test_gpu_crt import _check, _normal, product  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def up256(x):
+    return (x + 255) // 256 * 256
+
+
+# rows are halved first, to 384 of 520 and 256 of 330, below a number of columns that is no multiple of 16: the
+# scratch lies between 384 x 520 (256 x 330) bytes per modulus, which do not hold the block, and its padded columns'
+@pytest.mark.parametrize("m,n,mb,K", [(520, 520, 384, 64), (330, 330, 256, 72)])
+def test_crt_blocks_of_fewer_rows_than_columns(product, m, n, mb, K):  # noqa: F811
+    A, B = _normal(m, K), _normal(n, K, seed=2)
+    need = sum(up256(16 * r * K * 2) + up256(4 * r) for r in (mb, n)) + up256(16 * n * mb)
+    C = torch.empty(m, n, dtype=torch.float64, device="cuda")
+    _check(product(A, B, C, 1, 1, scratch=need), A, B)
