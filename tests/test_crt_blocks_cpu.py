@@ -1,7 +1,9 @@
 """Blocks of the FP64-class product (csrc/crt_gemm.cu) against its scratch: what
 every block lays out, counted here from the documented layout, fits, for any
-shape and any scratch down to the least one.  No device."""
+shape and any scratch down to the least one; and its K splits against the words
+of the reconstruction.  No device."""
 import ctypes
+import math
 import random
 
 import pytest
@@ -60,3 +62,23 @@ def test_every_scratch_down_to_the_least(lib):
         m, n = sorted((int(2 ** rng.uniform(0, 17)), int(2 ** rng.uniform(0, 17))), reverse=True)
         check(lib, m, n, int(2 ** rng.uniform(0, 18)), int(least * 2 ** rng.uniform(0, 8)) + 256)
     assert blocks(lib, 128, 16, 8192, least - 256) is None
+
+
+def test_splits_fit_the_reconstruction(lib):
+    """Residues of all K splits are summed before the reconstruction, which adds (sum of three moduli's) x (M / the
+    three) in 32-bit words held in 64 bits: no word may wrap at the most splits that any K and any GPU get."""
+    f = getattr(lib, "_ZN6ladder14crt_gemm_bytesExxxi")
+    f.restype, f.argtypes = ctypes.c_size_t, [ctypes.c_longlong] * 3 + [ctypes.c_int]
+    operands = block_need(1, 1, 1 << 20) - MODULI * 16
+    splits = (f(1, 1, 1 << 20, 1 << 20) - operands) // (MODULI * 16)
+    assert (f(1, 1, 64, 1 << 20) - (block_need(1, 1, 64) - MODULI * 16)) // (MODULI * 16) == 1 < splits
+    p = [256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193]
+    threes = [(0, 1, 2), (4, 5, 6), (8, 9, 10), (12, 13, 14), (3, 7, 11), (15,)]
+    for word in range(4):
+        total = 1 << 32  # carry
+        for t in threes:
+            q = math.prod(p[i] for i in t)
+            most = splits * sum((q // p[i]) * (p[i] - 1) for i in t)
+            assert most < 1 << 32
+            total += most * ((math.prod(p) // q >> (32 * word)) & 0xffffffff)
+        assert total < 1 << 64

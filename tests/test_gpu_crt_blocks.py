@@ -1,4 +1,4 @@
-"""The FP64-class product (csrc/crt_gemm.cu) in blocks of fewer rows than columns."""
+"""The FP64-class product (csrc/crt_gemm.cu) in blocks of fewer rows than columns and at its most K splits."""
 import pytest
 
 from test_gpu_crt import _check, _normal, product  # noqa: F401
@@ -19,3 +19,10 @@ def test_crt_blocks_of_fewer_rows_than_columns(product, m, n, mb, K):  # noqa: F
     need = sum(up256(16 * r * K * 2) + up256(4 * r) for r in (mb, n)) + up256(16 * n * mb)
     C = torch.empty(m, n, dtype=torch.float64, device="cuda")
     _check(product(A, B, C, 1, 1, scratch=need), A, B)
+
+
+# operands of one sign just below a power of two: residues' sums over 19 splits of K near their largest
+def test_crt_splits_of_one_sign(product):  # noqa: F811
+    A, B = 1.0 - _normal(3, 20000).abs() * 2.0 ** -40, 1.0 - _normal(9, 20000, seed=2).abs() * 2.0 ** -45
+    C = torch.empty(3, 9, dtype=torch.float64, device="cuda")
+    _check(product(A, B, C, 1, 1), A, B)
