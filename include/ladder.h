@@ -329,7 +329,7 @@ ladder_status ladder_backward(ladder_plan_t plan, const double *B, const double 
  * the same (o, v, naux) with its workspace set; its mode decides the ladder's
  * precision, LADDER_FP64 or LADDER_OZAKI for an FP64-class solution); every
  * other contraction is an FP64-class product on the tensor cores (exact
- * integer products of the operands rounded to 51 to 58 bits under the largest
+ * integer products of the operands rounded to 53 to 58 bits under the largest
  * element of their row; see csrc/crt_gemm.cu).  The residual is the
  * spin-orbital one (the projections of exp(-T) H exp(T) with the one- and
  * two-body intermediates of Stanton, Gauss, Watts and Bartlett 1991) with the

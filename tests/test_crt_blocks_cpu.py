@@ -60,8 +60,15 @@ def test_every_scratch_down_to_the_least(lib):
     least = block_need(128, 16, 8192)
     for _ in range(4000):
         m, n = sorted((int(2 ** rng.uniform(0, 17)), int(2 ** rng.uniform(0, 17))), reverse=True)
-        check(lib, m, n, int(2 ** rng.uniform(0, 18)), int(least * 2 ** rng.uniform(0, 8)) + 256)
+        check(lib, m, n, int(2 ** rng.uniform(0, 21)), int(least * 2 ** rng.uniform(0, 8)) + 256)
     assert blocks(lib, 128, 16, 8192, least - 256) is None
+
+
+def test_long_contractions_run_in_even_blocks(lib):
+    """At most 2^17 terms a block, which leaves 53 bits to the operands."""
+    for k in (1 << 17, (1 << 17) + 1, 300000, 1 << 20, (1 << 30) - 1):
+        kb = blocks(lib, 1, 1, k, 1 << 40)[2]
+        assert kb <= 1 << 17 and -(-k // kb) == -(-k // (1 << 17)) and min(58, (123 - (kb - 1).bit_length()) // 2) >= 53
 
 
 def test_splits_fit_the_reconstruction(lib):
@@ -69,8 +76,8 @@ def test_splits_fit_the_reconstruction(lib):
     three) in 32-bit words held in 64 bits: no word may wrap at the most splits that any K and any GPU get."""
     f = getattr(lib, "_ZN6ladder14crt_gemm_bytesExxxi")
     f.restype, f.argtypes = ctypes.c_size_t, [ctypes.c_longlong] * 3 + [ctypes.c_int]
-    operands = block_need(1, 1, 1 << 20) - MODULI * 16
-    splits = (f(1, 1, 1 << 20, 1 << 20) - operands) // (MODULI * 16)
+    operands = block_need(1, 1, 1 << 17) - MODULI * 16
+    splits = (f(1, 1, 1 << 17, 1 << 20) - operands) // (MODULI * 16)
     assert (f(1, 1, 64, 1 << 20) - (block_need(1, 1, 64) - MODULI * 16)) // (MODULI * 16) == 1 < splits
     p = [256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193]
     threes = [(0, 1, 2), (4, 5, 6), (8, 9, 10), (12, 13, 14), (3, 7, 11), (15,)]

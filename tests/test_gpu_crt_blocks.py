@@ -1,4 +1,5 @@
-"""The FP64-class product (csrc/crt_gemm.cu) in blocks of fewer rows than columns and at its most K splits."""
+"""The FP64-class product (csrc/crt_gemm.cu) in blocks of fewer rows than columns, at its most K splits
+and in blocks of K."""
 import pytest
 
 from test_gpu_crt import _check, _normal, product  # noqa: F401
@@ -26,3 +27,15 @@ def test_crt_splits_of_one_sign(product):  # noqa: F811
     A, B = 1.0 - _normal(3, 20000).abs() * 2.0 ** -40, 1.0 - _normal(9, 20000, seed=2).abs() * 2.0 ** -45
     C = torch.empty(3, 9, dtype=torch.float64, device="cuda")
     _check(product(A, B, C, 1, 1), A, B)
+
+
+# more than 2^17 terms: the operands' last bit, 2^-53 below the power of two above their row, decides the result
+@pytest.mark.parametrize("K", [1 << 17, (1 << 17) + 2, 500000])
+def test_crt_long_contractions_keep_53_bits(product, K):  # noqa: F811
+    sign = torch.ones(K, dtype=torch.float64, device="cuda")
+    sign[1::2] = -1.0
+    A = (0.75 + 2.0 ** -53 * (sign > 0).double())[None].repeat(2, 1)
+    assert A.dtype == torch.float64
+    B = (0.75 * sign)[None].repeat(3, 1)
+    C = product(A, B, torch.empty(2, 3, dtype=torch.float64, device="cuda"), 1, 1)
+    assert bool((C == K // 2 * 0.75 * 2.0 ** -53).all())
