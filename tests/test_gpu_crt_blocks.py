@@ -1,5 +1,5 @@
-"""The FP64-class product (csrc/crt_gemm.cu) in blocks of fewer rows than columns, at its most K splits
-and in blocks of K."""
+"""The FP64-class product (csrc/crt_gemm.cu) in blocks of fewer rows than columns, at its most K splits,
+in blocks of K, and with rows down to the least numbers."""
 import pytest
 
 from test_gpu_crt import _check, _normal, product  # noqa: F401
@@ -39,3 +39,17 @@ def test_crt_long_contractions_keep_53_bits(product, K):  # noqa: F811
     B = (0.75 * sign)[None].repeat(3, 1)
     C = product(A, B, torch.empty(2, 3, dtype=torch.float64, device="cuda"), 1, 1)
     assert bool((C == K // 2 * 0.75 * 2.0 ** -53).all())
+
+
+def test_crt_rows_near_the_least_numbers(product):  # noqa: F811
+    """Rows near 2^-1022 keep their relative accuracy, and rows of subnormal numbers are exact."""
+    A, B = _normal(20, 100), _normal(30, 100, seed=2)
+    C = product(A, B, torch.empty(20, 30, dtype=torch.float64, device="cuda"), 1, 1)
+    for e in (-920, -1000):
+        tiny = A * 2.0 ** -500 * 2.0 ** (e + 500)
+        S = product(tiny, B * 2.0 ** 950, torch.empty_like(C), 1, 1)
+        assert torch.equal(S, C * 2.0 ** (e + 950))
+    whole = torch.round(A * 2.0 ** 45)
+    C = product(whole, B, torch.empty_like(C), 1, 1)
+    S = product(whole * 2.0 ** -600 * 2.0 ** -474, B * 2.0 ** 950, torch.empty_like(C), 1, 1)
+    assert torch.equal(S, C * 2.0 ** -124)
