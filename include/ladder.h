@@ -72,8 +72,9 @@ typedef enum {
  * (16 residues, Chinese remainder theorem) and are rounded once to FP64.  R has
  * a relative error of about 1e-16, below that of sums in FP64 (1e-15 and more).
  * B or tau with a NaN, an infinity or a magnitude of 2^300 and more, and shapes
- * whose scratch would exceed 64 GiB (v above about 570 at N = 4 v), run in FP64
- * arithmetic on the FP64 units instead.
+ * whose scratch would exceed 64 GiB (v above about 570 at N = 4 v) or is given
+ * smaller (ladder_workspace_least), run in FP64 arithmetic on the FP64 units
+ * instead.
  *
  * LADDER_OZAKI follows the error-free splitting of Ozaki, Ogita, Oishi and
  * Rump (Numer. Algorithms 59, 2012) on the BF16 tensor cores.  Each operand
@@ -205,8 +206,14 @@ ladder_status ladder_set_tile_range(ladder_plan_t plan, int tile_lo, int tile_hi
 /* Bytes of device scratch the plan needs (slices of B and tau, packed pair
  * combinations, reduction partials, the device status word).  The caller
  * allocates it and hands it over with ladder_set_workspace; the plan keeps
- * the pointer (not the memory) until ladder_destroy or the next call. */
+ * the pointer (not the memory) until ladder_destroy or the next call.
+ * Where memory is short, any size down to ladder_workspace_least is taken as
+ * well: an LADDER_FP64 plan with less than ladder_workspace_size runs in FP64
+ * arithmetic on the FP64 units, without the residues: less memory and slower
+ * (o=10, v=120, N=480: 2.6 GB and 4.6 ms, or 7 MB and 165 ms), and a plan LADDER_WITH_DRESSING
+ * dresses in smaller blocks; other plans have one size. */
 ladder_status ladder_workspace_size(ladder_plan_t plan, size_t *bytes);
+ladder_status ladder_workspace_least(ladder_plan_t plan, size_t *bytes);
 ladder_status ladder_set_workspace(ladder_plan_t plan, void *dptr, size_t bytes);
 
 /* Eq. pp-Ladder-01: tau = t2 + t1 (x) t1 on the device, in FP64.  tau may not alias t2. */
@@ -261,7 +268,7 @@ ladder_status ladder_apply_dressed(ladder_plan_t plan, const double *B, const do
  * products of operands rounded to at least 53 bits under their largest
  * element, one rounding to FP64 per element of W; NaN if one of its bounded
  * device waits runs out), in FP64 on the CUDA cores where its workspace would
- * exceed 128 GiB, and the energy terms in FP64; LADDER_TRIPLES_FP32 forms the
+ * exceed 128 GiB or is given smaller (below), and the energy terms in FP64; LADDER_TRIPLES_FP32 forms the
  * integrals and W in FP32 (the energy sums stay FP64), both on the CUDA cores;
  * LADDER_TRIPLES_BF16X6 forms the integrals in FP32 and runs the W contractions
  * on the tensor cores (tcgen05) as split-BF16 GEMMs: three BF16 slices of each
@@ -272,12 +279,17 @@ ladder_status ladder_apply_dressed(ladder_plan_t plan, const double *B, const do
  * supplies a workspace of at least ladder_triples_workspace_size bytes
  * (256-byte aligned): the integrals (o v^3 + o^3 v + o^2 v^2 elements), their
  * slices or residues on the tensor cores (FP64: 64 bytes per element of
- * o v^3), W of a batch of triples and the reduction partials.  Asynchronous on
- * `stream`; the result is reduced in a fixed order (bitwise reproducible). */
+ * o v^3), W of a batch of triples and the reduction partials.  FP64 takes less
+ * as well, down to ladder_triples_workspace_least (32 bytes per element of
+ * o v^3 in all), and then runs on the CUDA cores (o=8, v=60, N=240: 0.31 GB and
+ * 3.1 ms, or 0.06 GB and 53 ms).
+ * Asynchronous on `stream`; the result is reduced in a fixed order (bitwise
+ * reproducible). */
 #define LADDER_TRIPLES_FP64 0
 #define LADDER_TRIPLES_FP32 1
 #define LADDER_TRIPLES_BF16X6 2
 ladder_status ladder_triples_workspace_size(int o, int v, int naux, int precision, size_t *bytes);
+ladder_status ladder_triples_workspace_least(int o, int v, int naux, int precision, size_t *bytes);
 ladder_status ladder_triples(int o, int v, int naux, int precision, const double *B, const double *Bov,
                              const double *Boo, const double *t1, const double *t2, const double *e_occ,
                              const double *e_vir, double *E_dev, void *workspace, size_t ws_bytes,

@@ -29,9 +29,9 @@ STATUS = {0: "LADDER_OK", 1: "LADDER_EINVAL", 2: "LADDER_ENOMEM", 3: "LADDER_ECU
 # every entry point that include/ladder.h declares
 EXPORTS = ("ladder_plan", "ladder_plan_mode", "ladder_plan_shape", "ladder_ccsd_workspace_size", "ladder_ccsd",
            "ladder_get_tuning", "ladder_set_tuning", "ladder_tile_count",
-           "ladder_set_tile_range", "ladder_workspace_size", "ladder_set_workspace",
+           "ladder_set_tile_range", "ladder_workspace_size", "ladder_workspace_least", "ladder_set_workspace",
            "ladder_tau", "ladder_apply", "ladder_apply_dressed", "ladder_triples_workspace_size",
-           "ladder_triples", "ladder_energy", "ladder_energy_noalloc", "ladder_backward", "ladder_pair_combine", "ladder_apply_host",
+           "ladder_triples_workspace_least", "ladder_triples", "ladder_energy", "ladder_energy_noalloc", "ladder_backward", "ladder_pair_combine", "ladder_apply_host",
            "ladder_plan_batched", "ladder_set_member_tuning", "ladder_apply_batched", "ladder_step_batched", "ladder_last_device_error", "ladder_selftest_wait",
            "ladder_set_timing", "ladder_timing", "ladder_timing_passes", "ladder_timing_dressing", "ladder_timing_sym", "ladder_flops", "ladder_status_string",
            "ladder_destroy")
@@ -80,11 +80,13 @@ def load_library(path: str = LIB_PATH):
         "ladder_tile_count": [_P, ip],
         "ladder_set_tile_range": [_P, i, i],
         "ladder_workspace_size": [_P, ctypes.POINTER(sz)],
+        "ladder_workspace_least": [_P, ctypes.POINTER(sz)],
         "ladder_set_workspace": [_P, _P, sz],
         "ladder_tau": [_P, _P, _P, _P, _P],
         "ladder_apply": [_P, _P, _P, _P, _P],
         "ladder_apply_dressed": [_P, _P, _P, _P, _P, _P, _P],
         "ladder_triples_workspace_size": [i, i, i, i, ctypes.POINTER(sz)],
+        "ladder_triples_workspace_least": [i, i, i, i, ctypes.POINTER(sz)],
         "ladder_triples": [i, i, i, i] + [_P] * 9 + [sz, _P],
         "ladder_energy": [_P, _P, _P, _P, _P],
         "ladder_energy_noalloc": [i, i, _P, _P, _P, _P],
@@ -174,6 +176,23 @@ def ladder_workspace_size(plan) -> int:
     return n.value
 
 
+def ladder_workspace_least(plan) -> int:
+    n = ctypes.c_size_t()
+    _check("ladder_workspace_least", load_library().ladder_workspace_least(plan, ctypes.byref(n)))
+    return n.value
+
+
+def _workspace(size, least, device):
+    """A uint8 tensor of `size` bytes, or of `least` where the device has no room for that."""
+    import torch
+    try:
+        return torch.empty(max(size, 256), dtype=torch.uint8, device=device)
+    except torch.cuda.OutOfMemoryError:
+        if least >= size:
+            raise
+    return torch.empty(max(least, 256), dtype=torch.uint8, device=device)
+
+
 def ladder_set_workspace(plan, ws) -> None:
     _check("ladder_set_workspace",
            load_library().ladder_set_workspace(plan, _ptr(ws), ws.numel() * ws.element_size()))
@@ -245,6 +264,13 @@ def ladder_triples_workspace_size(o: int, v: int, naux: int, precision: int) -> 
     return n.value
 
 
+def ladder_triples_workspace_least(o: int, v: int, naux: int, precision: int) -> int:
+    n = ctypes.c_size_t()
+    _check("ladder_triples_workspace_least",
+           load_library().ladder_triples_workspace_least(o, v, naux, precision, ctypes.byref(n)))
+    return n.value
+
+
 def ladder_triples(o, v, naux, precision, B, B_ov, B_oo, t1, t2, e_occ, e_vir, E, ws, stream=None) -> None:
     _check("ladder_triples", load_library().ladder_triples(
         o, v, naux, precision, _ptr(B), _ptr(B_ov), _ptr(B_oo), _ptr(t1), _ptr(t2), _ptr(e_occ),
@@ -261,8 +287,8 @@ def triples(B, B_ov, B_oo, t1, t2, e_occ, e_vir, precision="fp64", workspace=Non
     o = t1.shape[0]
     prec = TRIPLES_PRECISION[precision]
     if workspace is None:
-        n = ladder_triples_workspace_size(o, v, naux, prec)
-        workspace = torch.empty(max(n, 256), dtype=torch.uint8, device=B.device)
+        workspace = _workspace(ladder_triples_workspace_size(o, v, naux, prec),
+                               ladder_triples_workspace_least(o, v, naux, prec), B.device)
     E = torch.empty((), dtype=torch.float64, device=B.device)
     ladder_triples(o, v, naux, prec, B, B_ov, B_oo, t1, t2, e_occ, e_vir, E, workspace)
     return E
@@ -417,8 +443,8 @@ class Ladder:
                 if "two_pass" in tuning and "ksplit" not in tuning:
                     t.ksplit = 0  # the plan's own block-pair split for the chosen form
                 ladder_set_tuning(self.plan, t)
-            n = ladder_workspace_size(self.plan)
-            self.workspace = torch.empty(max(n, 256), dtype=torch.uint8, device=self.device)
+            self.workspace = _workspace(ladder_workspace_size(self.plan), ladder_workspace_least(self.plan),
+                                        self.device)
             ladder_set_workspace(self.plan, self.workspace)
 
     @property

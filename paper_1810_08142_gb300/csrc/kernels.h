@@ -86,8 +86,9 @@ struct CrtOut {
 };
 // scratch that keeps an (m x K) by (n x K) product in one piece, or in blocks of
 // K of at most 2^17; less is enough (the product then runs in shorter blocks of
-// K, each added in FP64, and of rows), down to the figure for m = 128, n = 16, K = 8192
+// K, each added in FP64, and of rows), down to crt_gemm_least
 size_t crt_gemm_bytes(long long m, long long n, long long K, int sms);
+size_t crt_gemm_least(long long m, long long n, long long K, int sms);
 // rows, columns and K of the blocks that crt_gemm (m >= n) takes in this scratch; false: none fits
 bool crt_gemm_blocks(long long m, long long n, long long K, int sms, size_t scratch_bytes, long long (&blk)[3]);
 cudaError_t crt_init_attributes();  // once per device, outside stream capture
