@@ -1666,7 +1666,9 @@ cudaError_t launch_oz_xsym(const OzLaunch &L, int nslices, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// two blocks per SM, each walking the units
+// one block per SM, each walking the units in their order, so that the units under
+// way share integral tiles in L2 (two blocks per SM need 64 registers a thread and
+// spill: 418 -> 743 us at v = 120)
 cudaError_t launch_oz_vform(const OzLaunch &L, int nslices, int sm_count, cudaStream_t s) {
   if (L.nitems <= 0) return cudaSuccess;
   const int grid = std::min(L.nitems, sm_count);

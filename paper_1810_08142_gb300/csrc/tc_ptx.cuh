@@ -130,19 +130,11 @@ __device__ __forceinline__ void fence_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem desc] * B[smem desc]^T, bf16 inputs, fp32 accumulate.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// The same two for a whole warp in step, of which one elected lane issues.  In
-// code that all lanes run with values the compiler can see to be warp-uniform,
-// the operands stay in uniform registers, where the instruction takes them;
+// D[tmem] (+)= A[smem desc] * B[smem desc]^T, bf16 inputs, fp32 accumulate, and
+// an arrival on `bar` once all MMAs issued so far complete, for a whole warp in
+// step, of which one elected lane (always the same) issues.  In code that all
+// lanes run with values the compiler can see to be warp-uniform, the operands
+// stay in uniform registers, where the instruction takes them;
 // under `if (lane == 0)` they are moved there for every MMA, which kept the
 // kernels' issue at 75 to 100 clocks an MMA (50 this way): the error-free storing
 // pass of o = 16, v = 200 20.1 -> 17.1 ms, the GEMM2 pass of split-BF16 dB of the
@@ -163,13 +155,6 @@ __device__ __forceinline__ void mma_commit_warp(uint32_t bar) {
 }
 // a value that every lane holds, as one the compiler takes for warp-uniform
 __device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
-
-// Arrive on `bar` once all tcgen05.mma issued so far by this thread complete.
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-      : "memory");
-}
 
 // Each thread of the warp reads 16 consecutive 32-bit columns of its lane.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
@@ -194,18 +179,6 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&r)[4]) {
                : "memory");
 #pragma unroll
   for (int i = 0; i < 4; ++i) r[i] = __uint_as_float(u[i]);
-}
-// Each thread of the warp reads 8 consecutive 32-bit columns of its lane.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&r)[8]) {
-  uint32_t u[8];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]),
-        "=r"(u[7])
-      : "r"(taddr)
-      : "memory");
-#pragma unroll
-  for (int i = 0; i < 8; ++i) r[i] = __uint_as_float(u[i]);
 }
 // Each thread of the warp writes 16 consecutive 32-bit columns of its lane.
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&r)[16]) {
