@@ -67,10 +67,13 @@ typedef enum {
 } ladder_mode;
 
 /* LADDER_FP64 forms R from two FP64-class products on the tensor cores: every
- * operand row is rounded to 53 to 58 bits under its largest element (a slot of
- * V+- first weighed with its largest amplitude), the integer products are exact
- * (16 residues, Chinese remainder theorem) and are rounded once to FP64.  R has
- * a relative error of about 1e-16, below that of sums in FP64 (1e-15 and more).
+ * operand row is rounded to so many bits under its largest element (a slot of V+-
+ * first weighed with its largest amplitude), the integer products are exact (16
+ * residues, Chinese remainder theorem) and are rounded once to FP64.  The bits:
+ * 58 to 53 for B, by naux; 57 to 52 for tau+-, by v (54 from v = 113, 53 from 241,
+ * 52 from 497); one less than tau+-'s for the integrals that V+- is formed from.
+ * R has a relative error of 1e-16 at v = 60, 7e-16 at v = 200 and 3e-15 at v =
+ * 560, below that of FP64 sums (6e-15 at v = 200, 1.4e-14 at v = 560).
  * B or tau with a NaN, an infinity or a magnitude of 2^300 and more, and shapes
  * whose scratch would exceed 64 GiB (v above about 570 at N = 4 v) or is given
  * smaller (ladder_workspace_least), run in FP64 arithmetic on the FP64 units
@@ -209,9 +212,9 @@ ladder_status ladder_set_tile_range(ladder_plan_t plan, int tile_lo, int tile_hi
  * the pointer (not the memory) until ladder_destroy or the next call.
  * Where memory is short, any size down to ladder_workspace_least is taken as
  * well: an LADDER_FP64 plan with less than ladder_workspace_size runs in FP64
- * arithmetic on the FP64 units, without the residues: less memory and slower
- * (o=10, v=120, N=480: 2.6 GB and 4.6 ms, or 7 MB and 165 ms), and a plan LADDER_WITH_DRESSING
- * dresses in smaller blocks; other plans have one size. */
+ * arithmetic on the FP64 units, without the residues (o=10, v=120, N=480: 2.6 GB
+ * and 4.6 ms, or 7 MB and 165 ms), and a plan LADDER_WITH_DRESSING dresses in
+ * smaller blocks; other plans have one size. */
 ladder_status ladder_workspace_size(ladder_plan_t plan, size_t *bytes);
 ladder_status ladder_workspace_least(ladder_plan_t plan, size_t *bytes);
 ladder_status ladder_set_workspace(ladder_plan_t plan, void *dptr, size_t bytes);
@@ -222,11 +225,11 @@ ladder_status ladder_tau(ladder_plan_t plan, const double *t1, const double *t2,
 
 /* Eq. pp-Ladder-0: R_ij^ab = sum_cd (ac|bd) tau_ij^cd.  R is overwritten (not
  * accumulated); R may not alias B or tau.  The (ac|bd) integrals are formed
- * tile by tile on the tensor cores.  LADDER_FP64 and the fused split-BF16 form
- * (two_pass = 0) never write them to memory; the two-pass form (the split-BF16
- * default where it fits, and LADDER_OZAKI) writes their sliced symmetric and
- * antisymmetric combinations V+- to the workspace once and reads them back in
- * its GEMM2 pass. */
+ * tile by tile on the tensor cores.  The fused split-BF16 form (two_pass = 0)
+ * never writes them to memory; the two-pass form (the split-BF16 default where it
+ * fits, and LADDER_OZAKI) writes their sliced symmetric and antisymmetric
+ * combinations V+- to the workspace once and reads them back in its GEMM2 pass,
+ * and LADDER_FP64 writes the integrals and V+- of a block of a at a time. */
 ladder_status ladder_apply(ladder_plan_t plan, const double *B, const double *tau,
                            double *R, void *stream);
 
@@ -265,11 +268,13 @@ ladder_status ladder_apply_dressed(ladder_plan_t plan, const double *B, const do
  * 1 <= o <= 256, 1 <= v <= 1024, 1 <= naux <= 65536.
  * E_dev: one double (device memory).  precision LADDER_TRIPLES_FP64 forms the
  * integrals and W in FP64-class products on the tensor cores (exact integer
- * products of operands rounded to at least 53 bits under their largest
- * element, one rounding to FP64 per element of W; NaN if one of its bounded
- * device waits runs out), in FP64 on the CUDA cores where its workspace would
- * exceed 128 GiB or is given smaller (below), and the energy terms in FP64; LADDER_TRIPLES_FP32 forms the
- * integrals and W in FP32 (the energy sums stay FP64), both on the CUDA cores;
+ * products of operands rounded to at least 53 bits, the integrals' under the
+ * largest of their row and W's, 55 to 58, under the largest of all (ia|bd) and
+ * (ck|jl) and of all t2; one rounding to FP64 per element of W; NaN if one of its
+ * bounded device waits runs out), in FP64 on the CUDA cores where its workspace
+ * would exceed 128 GiB or is given smaller (below), and the energy terms in FP64;
+ * LADDER_TRIPLES_FP32 forms the integrals and W in FP32 (the energy sums stay
+ * FP64), both on the CUDA cores;
  * LADDER_TRIPLES_BF16X6 forms the integrals in FP32 and runs the W contractions
  * on the tensor cores (tcgen05) as split-BF16 GEMMs: three BF16 slices of each
  * FP32 operand, the six slice products p + q < 3, FP32 accumulation with the

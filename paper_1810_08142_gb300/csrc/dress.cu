@@ -28,7 +28,7 @@
 // there, so FP32 keeps it far inside their tolerance) and the FP32 and BF16X6
 // triples; the FP64 and error-free modes form all of these products on the
 // tensor cores instead (crt_gemm.cu), and T is double only for FP64 triples
-// too large for that.
+// too large for that or given the least workspace.
 #include <algorithm>
 #include <type_traits>
 

@@ -2,8 +2,9 @@
 // 1.1 TFLOP/s on this GPU).  It runs for inputs and shapes that the residue
 // products of crt_gemm.cu do not take: NaN, infinity or magnitudes of 2^300 and
 // more (both forms are launched, and this one returns at once where the input
-// is ordinary), and scratch above 64 GiB.  At every size measured the residue
-// form is faster: o=2, v=12, N=45 705 -> 75 us, o=10, v=120, N=480 165 -> 5.1 ms.
+// is ordinary), scratch above 64 GiB, and plans given less workspace than the
+// residues need.  At every size measured the residue form is faster: o=2, v=12,
+// N=45 705 -> 75 us, o=10, v=120, N=480 165 -> 4.7 ms.
 //
 // R_ij^ab = sum_cd (ac|bd) tau_ij^cd (Eq. pp-Ladder-0) with (ac|bd) =
 // sum_P B^P_ac B^P_bd (Eq. RIM), evaluated through the symmetric /

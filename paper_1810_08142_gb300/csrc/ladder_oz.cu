@@ -44,8 +44,8 @@
 // products of every 16-slot piece with p + q < S, issued and drained by order
 // group so that draining one group overlaps the MMAs of the other.  The unpack kernel of the two-pass form then writes R.
 //
-// Warp roles (576 threads): warp 0 TMA producer, warp 1 MMA issuer (one
-// thread), warps 2-17 conversion (four per TMEM lane quadrant, each owning a
+// Warp roles (576 threads): warp 0 TMA producer, warp 1 MMA issuer (in step, one
+// elected lane), warps 2-17 conversion (four per TMEM lane quadrant, each owning a
 // quarter of the columns).
 #include <algorithm>
 
