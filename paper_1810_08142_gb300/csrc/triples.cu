@@ -83,6 +83,11 @@ __global__ void __launch_bounds__(kTE) triples_energy_kernel(const TriplesArgs a
   auto singles = [&](int x, int y, int z) -> T {
     return Ijk[y * v + z] * sti[x] + Iik[x * v + z] * stj[y] + Iij[x * v + y] * stk[z];
   };
+  auto on_singles = [&](T s, int x, int y, int z) -> T {  // one multiply-add each
+    s += Ijk[y * v + z] * sti[x];
+    s += Iik[x * v + z] * stj[y];
+    return s + Iij[x * v + y] * stk[z];
+  };
   // the thread's sum: FP64 for T = double; for T = float a double-single
   // (hi, lo) kept with TwoSum on the FP32 pipe (about 48 bits), widened once
   double s = 0.0;
@@ -129,14 +134,20 @@ __global__ void __launch_bounds__(kTE) triples_energy_kernel(const TriplesArgs a
     // permutations, so that each w, V and integral is read once instead of up
     // to six times.  In FP64 they share D, and with the even permutations (abc,
     // bca, cab) and the odd ones (acb, bac, cba) the sum of their terms is
-    //   sum_p (3 w_p + sum of its parity's w) (3 V_p - sum of the other parity's V) / (3 D).
+    //   sum_p (3 w_p + sum of its parity's w) (3 V_p - sum of the other parity's V) / (3 D)
+    //     = (sum_p w_p r_p + (w_even - w_odd) (V_even - V_odd)) / D,  r_p the second factor
+    // (w_even and the like: sums), which knows w and V only up to a constant each: both
+    // are taken less the first one's.  Of i = j = k they agree in all permutations,
+    // and where one occupied orbital dominates what rounding leaves of its triple
+    // exceeds E(T) (with factors of 2^-5 and 2^-10 between the occupied orbitals
+    // errors of up to 1e-12 and 4e-8 with w and V as they are, 2e-16 so).
     // An orbit of two (one) distinct blocks visits every ordering twice (six
     // times).  At o = 10, v = 120 (FP32) 3.90 -> 1.8 ms in all, at o = 8, v = 60
     // (FP64, bound by the FP64 pipe) 3.44 -> 1.10 ms.
     const int X0 = A * kTC, Y0 = B * kTC, Z0 = C * kTC;
     const int c0 = cid & 15, c1 = (cid >> 4) & 15, c2 = (cid >> 8) & 15, c3 = (cid >> 12) & 15, c4 = (cid >> 16) & 15,
               c5 = cid >> 20;
-    const T third = n == 6 ? T(1) / T(3) : n == 3 ? T(1) / T(6) : T(1) / T(18);
+    const T share = n == 6 ? T(1) : n == 3 ? T(0.5) : T(1) / T(6);
 #pragma unroll
     for (int h = 0; h < kCube / kTE; ++h) {
       const int e = threadIdx.x + h * kTE;
@@ -145,9 +156,9 @@ __global__ void __launch_bounds__(kTE) triples_energy_kernel(const TriplesArgs a
       if (aa >= v || bb >= v || cc >= v) continue;
       const T w0 = cube[c0][al][bl][cl], w1 = cube[c1][bl][cl][al], w2 = cube[c2][cl][al][bl];
       const T w3 = cube[c3][al][cl][bl], w4 = cube[c4][bl][al][cl], w5 = cube[c5][cl][bl][al];
-      const T x0 = w0 + singles(aa, bb, cc), x1 = w1 + singles(bb, cc, aa), x2 = w2 + singles(cc, aa, bb);
-      const T x3 = w3 + singles(aa, cc, bb), x4 = w4 + singles(bb, aa, cc), x5 = w5 + singles(cc, bb, aa);
       if constexpr (std::is_same<T, float>::value) {
+        const T x0 = w0 + singles(aa, bb, cc), x1 = w1 + singles(bb, cc, aa), x2 = w2 + singles(cc, aa, bb);
+        const T x3 = w3 + singles(aa, cc, bb), x4 = w4 + singles(bb, aa, cc), x5 = w5 + singles(cc, bb, aa);
         // FP32: the six terms one by one, each rounded as it stands (their
         // common factors, taken out as below, would move E(T) by 3e-8)
         const float weight = n == 3 ? 0.5f : 1.f;  // n = 1: the first alone
@@ -170,14 +181,20 @@ __global__ void __launch_bounds__(kTE) triples_energy_kernel(const TriplesArgs a
           sh = x;
         }
       } else {
-        const T we = w0 + w1 + w2, wo = w3 + w4 + w5, xe = x0 + x1 + x2, xo = x3 + x4 + x5;
-        T t = (T(3) * w0 + we) * (T(3) * x0 - xo);
-        t += (T(3) * w1 + we) * (T(3) * x1 - xo);
-        t += (T(3) * w2 + we) * (T(3) * x2 - xo);
-        t += (T(3) * w3 + wo) * (T(3) * x3 - xe);
-        t += (T(3) * w4 + wo) * (T(3) * x4 - xe);
-        t += (T(3) * w5 + wo) * (T(3) * x5 - xe);
-        s += (double)(t * third / (eijk - sev[aa] - sev[bb] - sev[cc]));
+        const T v1 = w1 - w0, v2 = w2 - w0, v3 = w3 - w0, v4 = w4 - w0, v5 = w5 - w0;
+        // V minus the first one's
+        const T s0 = singles(aa, bb, cc);
+        const T y1 = on_singles(v1 - s0, bb, cc, aa), y2 = on_singles(v2 - s0, cc, aa, bb);
+        const T y3 = on_singles(v3 - s0, aa, cc, bb), y4 = on_singles(v4 - s0, bb, aa, cc);
+        const T y5 = on_singles(v5 - s0, cc, bb, aa);
+        const T ye = y1 + y2, yo = y3 + y4 + y5;
+        T t = (v1 + v2 - v3 - v4 - v5) * (ye - yo);
+        t += v1 * (T(3) * y1 - yo);
+        t += v2 * (T(3) * y2 - yo);
+        t += v3 * (T(3) * y3 - ye);
+        t += v4 * (T(3) * y4 - ye);
+        t += v5 * (T(3) * y5 - ye);
+        s += (double)(t * share / (eijk - sev[aa] - sev[bb] - sev[cc]));
       }
     }
   }  // orbits
