@@ -270,8 +270,8 @@ ladder_status ladder_apply_dressed(ladder_plan_t plan, const double *B, const do
  * integrals and W in FP64-class products on the tensor cores (exact integer
  * products of operands rounded to at least 53 bits, the integrals' under the
  * largest of their row and W's, 55 to 58, under the largest of all (ia|bd) and
- * (ck|jl) and of all t2; one rounding to FP64 per element of W; NaN if one of its
- * bounded device waits runs out), in FP64 on the CUDA cores where its workspace
+ * (ck|jl) and of all t2 times a weight of each of the row's orbitals; one rounding
+ * to FP64 per element of W; NaN if one of its bounded device waits runs out), in FP64 on the CUDA cores where its workspace
  * would exceed 128 GiB or is given smaller (below), and the energy terms in FP64;
  * LADDER_TRIPLES_FP32 forms the integrals and W in FP32 (the energy sums stay
  * FP64), both on the CUDA cores;

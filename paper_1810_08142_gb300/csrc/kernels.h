@@ -109,8 +109,8 @@ struct CrtSeg {
 // The triples' W[t][a][b][c] = sum over the six orderings of P, as three
 // residue products (one per virtual index that runs along the columns), each of
 // four K segments (two orderings, the d and the l contraction), into bytes
-// Y[modulus][t][a][b][cp]; all operands of one side share one scale, so the
-// residues of all orderings add up to W's.
+// Y[modulus][t][a][b][cp]; all operands of one side share one scale and the
+// weights of the orbitals, so the residues of all orderings add up to W's.
 struct CrtWArgs {
   CrtSeg seg[4];
   uint8_t *Y;
@@ -123,18 +123,30 @@ struct CrtWArgs {
   int col;                // the virtual index along the columns: 0 (a), 1 (b), 2 (c)
   unsigned long long timeout_ns;
 };
-// largest magnitude of n doubles as a bit pattern, by atomicMax into *out
-cudaError_t crt_absmax(const double *x, long long n, unsigned long long *out, cudaStream_t s);
-// residues of a whole view under the scale of max(*g0, *g1), `bits` bits;
-// first: as the first operand of a product (with the reconstruction's factors)
-cudaError_t crt_slice_shared(const CrtView &v, bool first, __nv_bfloat16 *out, const unsigned long long *g0,
-                             const unsigned long long *g1, int bits, cudaStream_t s);
-cudaError_t launch_crt_w(const CrtWArgs &a, int sms, cudaStream_t s);
-// W[t][abc] of nt triples from three Y arrays at distance `plane3`; the
-// operands' scales from max(*gA0, *gA1) and *gB
-cudaError_t launch_crt_w_finish(const uint8_t *Y, size_t plane3, int v, int cp, int nt, const unsigned long long *gA0,
-                                const unsigned long long *gA1, const unsigned long long *gB, int bits, double *W,
+constexpr int kTriplesMaxV = 1024;  // ladder_triples: v at most this (shared-memory vectors of its kernels)
+// Scales of the triples' operands: the largest |(ia|bd)|, |(ck|jl)| and |t2| (gm,
+// bit patterns, zero before crt_triples_weights) and an exponent per orbital.
+struct CrtOrbits {
+  int o, v;
+  unsigned long long *gm;
+  // scratch: exponents of the rows (i; b, a) of the integrals over d, (x; alpha,
+  // beta) of t2 over l, (z, y; c) of (ck|jl) over l and of t2 over d
+  int *ra, *rt, *rq, *rb;
+  int *u, *w;         // exponents of the virtual and occupied orbitals
+  int *uu, *wp, *wt;  // and u_a + u_b, w_z + w_y, and w_i + w_j + w_k of the sorted triples
+};
+// from ovvv[i][b][a][d], Q[z][y][c][l] and t2[z][y][c][d]
+cudaError_t crt_triples_weights(const CrtOrbits &a, const double *ovvv, const double *Q, const double *t2,
                                 cudaStream_t s);
+// residues of a whole view under the scale of max(*g0, *g1) times 2^ the weights
+// rw of its row's indices, `bits` bits; first: as the first operand of a product
+// (with the reconstruction's factors)
+cudaError_t crt_slice_shared(const CrtView &v, bool first, __nv_bfloat16 *out, const unsigned long long *g0,
+                             const unsigned long long *g1, const int *const (&rw)[3], int bits, cudaStream_t s);
+cudaError_t launch_crt_w(const CrtWArgs &a, int sms, cudaStream_t s);
+// W[t][abc] of the nt triples from t0 on, from three Y arrays at distance `plane3`
+cudaError_t launch_crt_w_finish(const uint8_t *Y, size_t plane3, int cp, int t0, int nt, const CrtOrbits &o, int bits,
+                                double *W, cudaStream_t s);
 
 // The ladder of an FP64 plan from residue products.  gmax: largest magnitudes
 // of B and of T+-, zero before the call; where one is at or above
@@ -152,7 +164,6 @@ size_t crt_ladder_bytes(int o, int v, int N, int K, int sms);
 cudaError_t crt_ladder(const CrtLadderArgs &a, cudaStream_t s);
 
 // ---- perturbative triples (triples.cu); W from launch_gemm with kEpiAcc3
-constexpr int kTriplesMaxV = 1024;  // ladder_triples: v at most this (shared-memory vectors of the energy kernel)
 struct TriplesArgs {
   const void *oovv;  // [j][k][b][c] = v_jk^bc = (bj|ck), element type T of the energy kernel
   const double *t1, *e_occ, *e_vir;

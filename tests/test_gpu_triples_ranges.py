@@ -3,7 +3,8 @@
 The factors and amplitudes carry a scale per orbital.  With one dominant occupied
 orbital its own triple vanishes (W and V are symmetric then), so E(T) comes from
 terms that lie the scale of the next orbital below those of that triple, which
-have to cancel.  The reference evaluates E(T) in numpy's extended type (64 bits of
+have to cancel, and the residues of W have to keep the bits of small operands.  The
+reference evaluates E(T) in numpy's extended type (64 bits of
 mantissa or more).
 
 Tolerance: W rounded once, about 20 FP64 operations per term and sums of terms of
@@ -34,7 +35,7 @@ def reference(B, Bov, Boo, t1, t2, e_occ, e_vir):
     return float((Z * (V - np.transpose(V, (0, 1, 2, 5, 4, 3))) / (3 * D)).sum())
 
 
-@pytest.mark.parametrize("bits", [0, 3, 5])
+@pytest.mark.parametrize("bits", [0, 3, 5, 10, 20, 30])
 @pytest.mark.parametrize("flat_t2", [False, True])
 @pytest.mark.parametrize("singles", [0.0, 0.01])
 def test_wide_orbital_ranges(bits, flat_t2, singles):
@@ -60,3 +61,22 @@ def test_wide_orbital_ranges(bits, flat_t2, singles):
         E = lad.triples(*[to_dev(x) for x in (B, Bov, Boo, t1, t2, e_occ, e_vir)]).item()
         E_ref = reference(B, Bov, Boo, t1, t2, e_occ, e_vir)
         assert abs(E - E_ref) <= 1e-13 * abs(E_ref), (seed, E, E_ref)
+
+def test_orbitals_without_integrals_or_amplitudes():
+    """Rows of zeros: an occupied and a virtual orbital without coupling leave E(T) of the others (to the order of its sum)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1810_08142_gb300 as lad
+    import synthetic
+    x = synthetic.make_inputs(3, 9, 12, 5)
+    E = lad.triples(*[to_dev(a) for a in (x.B, x.B_ov, x.B_oo, x.t1, x.t2, x.e_occ, x.e_vir)]).item()
+    z = synthetic.make_inputs(4, 10, 12, 5)
+    for name in ("B", "B_ov", "B_oo", "t1", "t2"):
+        a, b = getattr(z, name), getattr(x, name)
+        a[...] = 0.0
+        a[tuple(slice(0, k) for k in b.shape)] = b
+    z.e_occ[:3], z.e_vir[:9] = x.e_occ, x.e_vir
+    E2 = lad.triples(*[to_dev(a) for a in (z.B, z.B_ov, z.B_oo, z.t1, z.t2, z.e_occ, z.e_vir)]).item()
+    assert abs(E2 - E) <= 1e-14 * abs(E)
+    zero = [np.zeros_like(a) for a in (z.B, z.B_ov, z.B_oo, z.t1, z.t2)] + [z.e_occ, z.e_vir]
+    assert lad.triples(*[to_dev(a) for a in zero]).item() == 0.0
