@@ -95,9 +95,13 @@ cudaError_t crt_init_attributes();  // once per device, outside stream capture
 // a row of an operand with a NaN or an infinity makes its row (column) of C NaN
 cudaError_t crt_gemm(const CrtView &A, const CrtView &B, const CrtOut &C, double alpha, double beta, void *scratch,
                      size_t scratch_bytes, int *status, int sms, cudaStream_t s);
-// or what the FP64 sums give there; no operand may change before the product is complete
-cudaError_t crt_gemm_ieee(const CrtView &A, const CrtView &B, const CrtOut &C, double alpha, double beta, void *scratch,
-                          size_t scratch_bytes, int *status, int sms, cudaStream_t s);
+// or what the FP64 sums give there; no operand may change before the product is
+// complete.  kx (nullable): an exponent per index of K; A is rounded as 2^-kx A
+// and B as 2^kx B, so that elements which meet small ones may be large
+cudaError_t crt_gemm_ieee(const CrtView &A, const CrtView &B, const CrtOut &C, double alpha, double beta, const int *kx,
+                          void *scratch, size_t scratch_bytes, int *status, int sms, cudaStream_t s);
+// such exponents from A [M][K]: 2^kx just above its largest element at that index
+cudaError_t crt_kslots(const double *A, int M, int K, int *kx, cudaStream_t s);
 // 4-D tensor map [planes][groups][rows][cols] of BF16, boxes (box_cols, box_rows) with 128-byte swizzle
 bool encode_bf16_rows(CUtensorMap *m, void *base, uint64_t cols, uint64_t rows, uint64_t groups, uint64_t planes,
                       uint32_t box_cols, uint32_t box_rows);
