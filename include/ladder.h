@@ -72,8 +72,8 @@ typedef enum {
  * residues, Chinese remainder theorem) and are rounded once to FP64.  The bits:
  * 58 to 53 for B, by naux; 57 to 52 for tau+-, by v (54 from v = 113, 53 from 241,
  * 52 from 497); one less than tau+-'s for the integrals that V+- is formed from.
- * R has a relative error of 1e-16 at v = 60, 7e-16 at v = 200 and 3e-15 at v =
- * 560, below that of FP64 sums (6e-15 at v = 200, 1.4e-14 at v = 560).
+ * R has a relative error (of its norm) of 1e-16 at v = 60, 7e-16 at v = 200 and
+ * 3e-15 at v = 560, below that of FP64 sums (6e-15 at v = 200, 1.4e-14 at v = 560).
  * B or tau with a NaN, an infinity or a magnitude of 2^300 and more, and shapes
  * whose scratch would exceed 64 GiB (v above about 570 at N = 4 v) or is given
  * smaller (ladder_workspace_least), run in FP64 arithmetic on the FP64 units
